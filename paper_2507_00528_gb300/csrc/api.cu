@@ -69,7 +69,7 @@ void free_workspace(gnep_nlist* nl) {
   nl->ws_pairs[0] = nl->ws_pairs[1] = -1;
 }
 
-int alloc_workspace(gnep_model* m, gnep_nlist* nl) {
+int alloc_workspace(gnep_model* m, gnep_nlist* nl, cudaStream_t st) {
   if (nl->ws_mem && nl->ws_pairs[0] >= nl->L[0].n && nl->ws_pairs[1] >= nl->L[1].n) return GNEP_OK;
   free_workspace(nl);
   const Shape& s = m->shape;
@@ -99,7 +99,6 @@ int alloc_workspace(gnep_model* m, gnep_nlist* nl) {
   for (auto& it : items) total += align256(it.bytes);
   char* base = nullptr;
   GNEP_CUDA(cudaMalloc(&base, total));
-  GNEP_CUDA(cudaMemset(base, 0, total));
   size_t off = 0;
   for (auto& it : items) {
     *it.p = base + off;
@@ -108,6 +107,8 @@ int alloc_workspace(gnep_model* m, gnep_nlist* nl) {
   nl->ws_mem = base;
   nl->ws_pairs[0] = (int64_t)PR;
   nl->ws_pairs[1] = (int64_t)PA;
+  // on the stream of the kernels that fill it (a non-blocking one does not wait for the legacy stream)
+  GNEP_CUDA(cudaMemsetAsync(base, 0, total, st));
   return GNEP_OK;
 }
 
@@ -186,6 +187,8 @@ int gnep_create(gnep_model** out, int n_species, const int* species_z, double rc
   cudaMemset(m->grad, 0, 8 * n);
   cudaMemset(m->step, 0, sizeof(long long));
   if ((e = cudaMemset(m->err, 0, 3 * sizeof(int))) != cudaSuccess) return fail(e, "init");
+  // the copies and clears above are on the legacy stream, which non-blocking streams do not wait for
+  if ((e = cudaStreamSynchronize(nullptr)) != cudaSuccess) return fail(e, "init");
   *out = m;
   return GNEP_OK;
 }
@@ -292,7 +295,7 @@ static int finish_build(gnep_model* m, gnep_nlist* nl, const gnep_batch* b, cuda
   bool types_changed = false;
   if ((rc = build_lists(m, nl, b, st, &types_changed))) return rc;
   if (types_changed && (rc = run_species_perm(nl, st))) return rc;
-  if ((rc = alloc_workspace(m, nl))) return rc;
+  if ((rc = alloc_workspace(m, nl, st))) return rc;
   if (!nl->ready_ev) GNEP_CUDA(cudaEventCreateWithFlags(&nl->ready_ev, cudaEventDisableTiming));
   if (!nl->side) {  // created here, outside any stream capture
     GNEP_CUDA(cudaStreamCreateWithFlags(&nl->side, cudaStreamNonBlocking));
@@ -306,7 +309,7 @@ static int finish_build(gnep_model* m, gnep_nlist* nl, const gnep_batch* b, cuda
     GNEP_CUDA(cudaStreamSynchronize(st));
   }
   if (herr & kErrRevMissing) {
-    GNEP_CUDA(cudaMemset(m->err, 0, sizeof(int)));
+    GNEP_CUDA(cudaMemsetAsync(m->err, 0, sizeof(int), st));
     return set_error(GNEP_ERR_INVALID_ARG, "neighbour lists are not symmetric (internal error)");
   }
   return GNEP_OK;
@@ -913,6 +916,7 @@ int gnep_load(gnep_model* m, const char* path) {
   GNEP_CUDA(cudaMemcpy(m->adam_v, vv.data(), 4 * n, cudaMemcpyHostToDevice));
   GNEP_CUDA(cudaMemcpy(m->scale, sc.data(), 4 * d, cudaMemcpyHostToDevice));
   GNEP_CUDA(cudaMemcpy(m->step, &stp, sizeof(long long), cudaMemcpyHostToDevice));
+  GNEP_CUDA(cudaDeviceSynchronize());  // a copy may return before its last bytes have arrived
   return GNEP_OK;
 }
 
@@ -1018,7 +1022,7 @@ int gnep_sync_status(gnep_model* m, void* stream) {
   GNEP_CUDA(cudaGetLastError());
   int flag = 0;
   GNEP_CUDA(cudaMemcpy(&flag, m->err, sizeof(int), cudaMemcpyDeviceToHost));
-  if (flag) GNEP_CUDA(cudaMemset(m->err, 0, sizeof(int)));
+  if (flag) GNEP_CUDA(cudaMemsetAsync(m->err, 0, sizeof(int), st));
   if (flag & kErrNonFinite) return set_error(GNEP_ERR_NONFINITE, "loss was not finite; the update was skipped");
   if (flag & kErrTimeout) return set_error(GNEP_ERR_TIMEOUT, "a device-side wait gave up");
   if (flag & kErrRevMissing) return set_error(GNEP_ERR_INVALID_ARG, "neighbour lists are not symmetric (internal error)");

@@ -254,7 +254,7 @@ int run_scale(gnep_model* m, gnep_nlist* nl, cudaStream_t st);
 int run_species_perm(gnep_nlist* nl, cudaStream_t st);
 
 // Workspace sizing (api.cu).
-int alloc_workspace(gnep_model* m, gnep_nlist* nl);
+int alloc_workspace(gnep_model* m, gnep_nlist* nl, cudaStream_t st);
 void free_workspace(gnep_nlist* nl);
 
 // Stage profiler: when on, an event is recorded after every kernel launch of

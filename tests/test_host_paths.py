@@ -1,0 +1,105 @@
+"""The library's host side on a fake CUDA runtime (fake_cudart.cpp: device memory is
+host memory, kernels do not run), for what a GPU run cannot show safely: failed
+allocations, buffers of another GPU, and work that a call leaves on the legacy stream,
+which a non-blocking stream does not wait for.  Each test runs its body in a child
+process with the fake preloaded."""
+import os
+import subprocess
+import sys
+import textwrap
+
+import pytest
+
+from paper_2507_00528_gb300 import build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+PRELUDE = r"""
+import ctypes as C, struct, sys
+sys.path.insert(0, {root!r})
+from paper_2507_00528_gb300 import _lib
+L = _lib.load()
+fake = C.CDLL(None)
+for f in ("fake_plant", "fake_foreign", "fake_copies", "cudaMalloc"):
+    getattr(fake, f).argtypes = dict(fake_plant=[C.c_size_t, C.c_char_p], cudaMalloc=[C.c_void_p, C.c_size_t]).get(
+        f, [C.c_void_p])
+INVALID, OOM, CUDA = -1, -2, -3
+ST = C.c_void_p(0x1234)  # a stream that is not the legacy one
+
+def device(values, fmt):
+    # a device array of the values
+    raw = struct.pack("%d%s" % (len(values), fmt), *values)
+    p = C.c_void_p()
+    assert fake.cudaMalloc(C.byref(p), len(raw)) == 0
+    C.memmove(p, raw, len(raw))
+    return p.value
+
+def found(radial=40, angular=10, most=10, flags=16, err=0):
+    # what a build's search reports to the host next (BuildResult)
+    fake.fake_plant(32, struct.pack("qqiiii", radial, angular, most, flags, err, 0))
+
+def batch():
+    return _lib.Batch(1, 2, device([0, 2], "i"), device([1.0] * 6, "d"), device([0, 1], "i"),
+                      device([9.0, 0, 0, 0, 9.0, 0, 0, 0, 9.0], "d"))
+
+def model():
+    m = C.c_void_p()
+    assert L.gnep_create(C.byref(m), 2, None, 7.0, 4.0, 4, 4, 8, 8, 4, 0, 30, 0, 0) == 0
+    return m
+
+def built(m, b):
+    nl = C.c_void_p()
+    found()
+    assert L.gnep_build_neighbors(m, C.byref(b), C.byref(nl), ST) == 0, L.gnep_last_error()
+    return nl
+
+def labels():
+    return _lib.Labels(device([0.0], "d"), device([0.0] * 6, "f"), device([0.0] * 6, "d"), 1.0, 1.0, 0.1, 0.0, 0)
+"""
+
+
+@pytest.fixture(scope="session")
+def fake(tmp_path_factory):
+    build.build()
+    so = str(tmp_path_factory.mktemp("fake") / "libfake_cudart.so")
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I" + os.path.join(cuda, "include"),
+                    os.path.join(HERE, "fake_cudart.cpp"), "-o", so], check=True)
+    return so
+
+
+@pytest.fixture
+def run(fake):
+    def run(body):
+        code = PRELUDE.format(root=os.path.dirname(HERE)) + textwrap.dedent(body)
+        p = subprocess.run([sys.executable, "-c", code], env=dict(os.environ, LD_PRELOAD=fake), capture_output=True,
+                           text=True, timeout=120)
+        assert p.returncode == 0, p.stderr[-3000:]
+    return run
+
+
+def test_nothing_is_left_on_the_legacy_stream(run, tmp_path):
+    """Every call leaves its device work on its own stream, or has waited for it."""
+    run(f"""
+    m = model()
+    assert fake.fake_legacy_pending() == 0
+    b = batch()
+    nl = built(m, b)
+    assert fake.fake_legacy_pending() == 0
+    found(radial=4000, angular=1000)  # the lists and the workspace grow
+    before = fake.fake_memsets_on_streams()
+    assert L.gnep_rebuild_neighbors(m, C.byref(b), nl, ST) == 0
+    assert fake.fake_legacy_pending() == 0 and fake.fake_memsets_on_streams() >= before + 2
+    found(err=4)  # an asymmetric list, seen by the next molecular dynamics step
+    v = [device([0.0] * 6, "d") for _ in range(2)]
+    im, F = device([1.0, 1.0], "d"), device([0.0] * 6, "f")
+    assert L.gnep_md_verlet(m, nl, v[0], v[1], im, F, 1.0, None, ST) == INVALID
+    assert fake.fake_legacy_pending() == 0
+    fake.fake_plant(4, struct.pack("i", 1))  # a loss that was not finite
+    assert L.gnep_sync_status(m, ST) == -5
+    assert fake.fake_legacy_pending() == 0
+    fake.fake_plant(4, None)
+    path = {str(tmp_path / "m.ckpt")!r}.encode()
+    assert L.gnep_save(m, path) == 0 and L.gnep_load(m, path) == 0
+    assert fake.fake_legacy_pending() == 0
+    """)
