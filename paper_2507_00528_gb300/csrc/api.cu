@@ -247,11 +247,22 @@ int gnep_get_descriptor_scale(gnep_model* m, float* scale, int32_t n, void* stre
   return copy_out(scale, m->scale, 4 * (size_t)n, (cudaStream_t)stream);
 }
 
-static int check_nlist(const gnep_model* m, const gnep_nlist* nl) {
+static int check_shape(const gnep_model* m, const gnep_nlist* nl) {
   if (!m || !nl) return set_error(GNEP_ERR_INVALID_ARG, "NULL model or neighbour list");
   if (!(nl->shape == m->shape) || nl->rcr != m->rcr || nl->rca != m->rca)
     return set_error(GNEP_ERR_INVALID_ARG, "neighbour list was built for a model of another shape or cut-off");
   return GNEP_OK;
+}
+
+// A rebuild that failed midway leaves arrays of two batches, or none: only a rebuild takes such a list.
+static int check_built(const gnep_nlist* nl) {
+  return nl->built ? GNEP_OK
+                   : set_error(GNEP_ERR_INVALID_ARG, "the last build of this neighbour list failed; rebuild it first");
+}
+
+static int check_nlist(const gnep_model* m, const gnep_nlist* nl) {
+  const int rc = check_shape(m, nl);
+  return rc ? rc : check_built(nl);
 }
 
 // Orders the work that follows on `st` after the device work of the last
@@ -303,6 +314,7 @@ static int finish_build(gnep_model* m, gnep_nlist* nl, const gnep_batch* b, cuda
     GNEP_CUDA(cudaEventCreateWithFlags(&nl->join_ev, cudaEventDisableTiming));
   }
   GNEP_CUDA(cudaEventRecord(nl->ready_ev, st));
+  nl->built = true;
   int herr = b ? 0 : nl->last_err;
   if (wait) {
     GNEP_CUDA(cudaMemcpyAsync(&herr, m->err, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -375,7 +387,8 @@ int gnep_build_neighbors(gnep_model* m, const gnep_batch* b, gnep_nlist** out, v
 
 int gnep_rebuild_neighbors(gnep_model* m, const gnep_batch* b, gnep_nlist* nl, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
-  int rc = use_nlist(m, nl, st);
+  int rc = check_shape(m, nl);
+  if (!rc) rc = after_build(nl, st);
   if (rc) return rc;
   if (!b || b->n_struct != nl->n_struct || b->n_atoms != nl->n_atoms)
     return set_error(GNEP_ERR_INVALID_ARG, "rebuild needs the same structure and atom counts");
@@ -402,7 +415,8 @@ int gnep_nlist_export(const gnep_nlist* nl, int which, int32_t* off, int32_t* j,
   if (!nl || which < 0 || which > 1) return set_error(GNEP_ERR_INVALID_ARG, "bad list");
   cudaStream_t st = (cudaStream_t)stream;
   const PairList& P = nl->L[which];
-  int rc = after_build(nl, st);
+  int rc = check_built(nl);
+  if (!rc) rc = after_build(nl, st);
   if (rc) return rc;
   if ((rc = copy_out(off, P.off, sizeof(int) * ((size_t)nl->n_atoms + 1), st))) return rc;
   if (P.n == 0) return GNEP_OK;

@@ -94,7 +94,7 @@ struct gnep_nlist {
     int na[2] = {0, 0}, ch[2] = {0, 0}, cg_blocks = 0, net_blocks = 0, radial_lanes = 0, net_tile = 0, beside = 0;
   } tune;
   uint64_t gen = 0;  // bumped whenever lists or tiles change (captured graphs check it)
-  bool built = false;        // the list holds a batch
+  bool built = false;        // lists, species grouping and workspace belong to one batch (false after a failed build)
   int last_err = 0;          // the model's error flag as the last build's search saw it
   void* host_res = nullptr;  // pinned: what a build's search reports to the host
   cudaEvent_t ready_ev = nullptr;    // the end of the last build's device work (consumers wait on it)

@@ -1066,7 +1066,9 @@ int build_lists(gnep_model* m, gnep_nlist* nl, const gnep_batch* b, cudaStream_t
   for (int L = 0; L < 2; ++L)
     if (r.tot[L] >= (1LL << 31) - 1)
       return set_error(GNEP_ERR_NEIGHBOR_OVERFLOW, "pair count exceeds 32-bit indices; split the batch");
-  *types_changed = (r.flags & kTypesChanged) != 0;
+  // from here on the list changes: until finish_build has seen the end of it, no call takes it
+  *types_changed = !nl->built || (r.flags & kTypesChanged);  // an unfinished build may have left any grouping
+  nl->built = false;
   nl->last_err = r.err;
 
   for (int L = 0; L < 2; ++L) {
@@ -1109,7 +1111,6 @@ int build_lists(gnep_model* m, gnep_nlist* nl, const gnep_batch* b, cudaStream_t
     (void)launch_pdl(k_reverse, blocks_for(P.n, 256), 256, 0, st, P.n, (const int*)P.off, (const int*)P.j,
                      (const int*)P.owner, (const char4*)P.shift, P.rev, m->err);
   GNEP_CHECK_LAUNCH("k_reverse");
-  nl->built = true;
   return GNEP_OK;  // the reverse search sets kErrRevMissing, reported later
 }
 

@@ -103,3 +103,55 @@ def test_nothing_is_left_on_the_legacy_stream(run, tmp_path):
     assert L.gnep_save(m, path) == 0 and L.gnep_load(m, path) == 0
     assert fake.fake_legacy_pending() == 0
     """)
+
+
+def test_a_list_whose_rebuild_failed_is_refused_until_it_is_rebuilt(run):
+    """Each allocation of a rebuild that grows the lists fails in turn.  The first, the
+    scratch, comes before any change; after the others no call may use the arrays, and
+    the next rebuild groups the species again."""
+    run("""
+    m, b, y = model(), batch(), labels()
+    nl = built(m, b)
+    found(radial=4000, angular=1000)
+    fake.fake_fail_alloc(0)
+    assert L.gnep_rebuild_neighbors(m, C.byref(b), nl, ST) == 0
+    total = fake.fake_allocs()
+    assert total >= 12  # scratch, 3 + 5 pair arrays, 2 for the grouping, the workspace
+    F = device([0.0] * 6, "f")
+    pos, vel, im = device([1.0] * 6, "d"), device([0.0] * 6, "d"), device([1.0, 1.0], "d")
+    off = (C.c_int32 * 3)()
+    g = C.c_void_p()
+    sched = (1e-3, 1e-6, 10, 100, 0.9, 0.999, 1e-8, 0.0)
+    def calls(nl):
+        return [L.gnep_forward(m, nl, None, None, F, None, ST), L.gnep_loss(m, nl, C.byref(y), None, ST),
+                L.gnep_loss_grad(m, nl, C.byref(y), None, None, ST), L.gnep_descriptors(m, nl, None, ST),
+                L.gnep_descriptors_noalloc(m, nl, device([0.0] * 50, "f"), ST),
+                L.gnep_nlist_export(nl, 0, off, None, None, ST),
+                L.gnep_compute_descriptor_scale(m, nl, ST),
+                L.gnep_graph_create(m, nl, C.byref(y), None, *(C.c_double(x) if isinstance(x, float) else x
+                                                               for x in sched), ST, C.byref(g))]
+    for nth in range(1, total + 1):
+        nl = built(m, b)
+        found(radial=4000, angular=1000)
+        fake.fake_fail_alloc(nth)
+        assert L.gnep_rebuild_neighbors(m, C.byref(b), nl, ST) == OOM, nth
+        fake.fake_fail_alloc(0)
+        n = fake.fake_launches()
+        if nth == 1:
+            assert calls(nl) == [0] * 8
+        else:
+            assert calls(nl) == [INVALID] * 8, nth
+            assert L.gnep_md_verlet(m, nl, pos, vel, im, F, 1.0, None, ST) == INVALID
+            assert fake.fake_launches() == n  # nothing ran on the broken list
+        fake.fake_fail_alloc(0)
+        found(radial=4000, angular=1000, flags=0)  # the same species as the failed batch
+        n = fake.fake_launches()
+        assert L.gnep_rebuild_neighbors(m, C.byref(b), nl, ST) == 0
+        regrouped = fake.fake_launches() - n
+        n = fake.fake_launches()
+        assert L.gnep_rebuild_neighbors(m, C.byref(b), nl, ST) == 0
+        assert regrouped - (fake.fake_launches() - n) == (0 if nth == 1 else 3), nth
+        assert calls(nl) == [0] * 8
+        assert L.gnep_md_verlet(m, nl, pos, vel, im, F, 1.0, None, ST) == 0
+        L.gnep_nlist_destroy(nl)
+    """)
