@@ -152,7 +152,7 @@ int gnep_build_neighbors(gnep_model *m, const gnep_batch *b, gnep_nlist **out,
  * rest of the build (compaction, reverse entries) queued on
  * `stream`: every call that reads `nl` afterwards, on any stream, is ordered
  * after that work by an event the list keeps.  The batch's arrays may be reused
- * once this returns; a batch that is refused leaves the lists as they were.  A rebuild that
+ * once this returns; a batch that is refused leaves the lists, and graphs captured on them, as they were.  A rebuild that
  * fails on the way (OOM, CUDA) leaves a list that every other call refuses with INVALID_ARG
  * until a rebuild of it succeeds.  The lists' internal consistency check of the
  * queued work is reported by gnep_sync_status() (or by the next

@@ -480,6 +480,7 @@ int gnep_md_verlet(gnep_model* m, gnep_nlist* nl, double* pos, double* vel, cons
     return set_error(GNEP_ERR_INVALID_ARG, "md: pos, vel, inv_mass and F must be device arrays");
   if (!(dt > 0.0)) return set_error(GNEP_ERR_INVALID_ARG, "md: dt must be positive");
   cudaStream_t st = (cudaStream_t)stream;
+  ++nl->gen;  // the list's positions move
   if ((rc = md_kick_drift(nl, pos, vel, inv_mass, F, dt, st))) return rc;  // leaves the positions in the list too
   if ((rc = finish_build(m, nl, nullptr, st, false))) return rc;           // lists for the new positions
   StepArgs A{m, nl, st};

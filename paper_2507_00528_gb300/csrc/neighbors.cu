@@ -1060,12 +1060,12 @@ int build_lists(gnep_model* m, gnep_nlist* nl, const gnep_batch* b, cudaStream_t
   if (r.flags & kBadOrder)
     return set_error(GNEP_ERR_INVALID_ARG, "struct_off must be strictly increasing (every structure holds an atom)");
   if (r.flags & kBadType) return set_error(GNEP_ERR_INVALID_ARG, "species index out of range");
-  ++nl->gen;  // graphs captured on the list no longer launch
   if (r.flags & kUnwrapped)
     return set_error(GNEP_ERR_INVALID_ARG, "positions must be wrapped into their cell (fractional coordinates in [0,1))");
   for (int L = 0; L < 2; ++L)
     if (r.tot[L] >= (1LL << 31) - 1)
       return set_error(GNEP_ERR_NEIGHBOR_OVERFLOW, "pair count exceeds 32-bit indices; split the batch");
+  ++nl->gen;  // graphs captured on the list no longer launch
   // from here on the list changes: until finish_build has seen the end of it, no call takes it
   *types_changed = !nl->built || (r.flags & kTypesChanged);  // an unfinished build may have left any grouping
   nl->built = false;

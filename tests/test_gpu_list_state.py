@@ -1,10 +1,14 @@
-"""Lists over rebuilds: a rebuild on a side stream into a batch with many more pairs (lists
-and workspace grow), evaluated at once on that stream, against a list built anew."""
+"""What a list and the graphs captured on it keep over rebuilds: a rebuild on a side
+stream into a batch with many more pairs (lists and workspace grow), evaluated at once
+on that stream, against a list built anew; and training graphs over rebuilds that are
+refused."""
 import numpy as np
 import pytest
 import torch
 
 from paper_2507_00528_gb300 import gnep, synth
+
+from gpu_common import Case, small_cells_batch
 
 pytestmark = pytest.mark.gpu
 
@@ -36,3 +40,31 @@ def test_growing_rebuild_on_a_side_stream():
         for out in (got, again):
             for x, y in zip(out, want):
                 assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("what", ["ends", "order", "type", "wrap", "nan"])
+def test_training_graph_outlives_a_refused_rebuild(what):
+    b = small_cells_batch()
+    c = Case("nmax4_basis8_h30", b)
+    sched = dict(lr_start=1e-3, lr_stop=1e-6, n_warmup=10, n_total=100)
+    g = gnep.TrainGraph(c.m, c.nl, c.gpu_labels(), **sched)
+    off, pos, typ = b.struct_off.copy(), b.pos.copy(), b.types.copy()
+    if what == "ends":
+        off[-1] -= 1
+    elif what == "order":
+        off[1] = off[2]
+    elif what == "type":
+        typ[5] = 7
+    else:
+        pos[3] = 100.0 if what == "wrap" else np.nan
+    bad = synth.Batch(off, pos, typ, b.cell)
+    with pytest.raises(gnep._lib.GnepError, match="INVALID_ARG"):
+        c.nl.rebuild(gnep.DeviceBatch.from_host(bad))
+    g.launch()
+    d = Case("nmax4_basis8_h30", b)
+    h = gnep.TrainGraph(d.m, d.nl, d.gpu_labels(), **sched)
+    h.launch()
+    assert torch.equal(g.loss, h.loss) and torch.equal(c.m.get_params(), d.m.get_params())
+    c.nl.rebuild(gnep.DeviceBatch.from_host(b))
+    with pytest.raises(gnep._lib.GnepError, match="rebuilt or retuned"):
+        g.launch()

@@ -155,3 +155,33 @@ def test_a_list_whose_rebuild_failed_is_refused_until_it_is_rebuilt(run):
         assert L.gnep_md_verlet(m, nl, pos, vel, im, F, 1.0, None, ST) == 0
         L.gnep_nlist_destroy(nl)
     """)
+
+
+def test_a_refused_batch_leaves_captured_graphs(run):
+    """Each refusal of a rebuild leaves the list as it was, so that graphs captured on it
+    still launch; a rebuild that went through, or a molecular dynamics step that moved the
+    list's positions, ends them."""
+    run("""
+    m, b, y = model(), batch(), labels()
+    nl = built(m, b)
+    def graph():
+        g = C.c_void_p()
+        assert L.gnep_graph_create(m, nl, C.byref(y), None, 1e-3, 1e-6, 10, 100, 0.9, 0.999, 1e-8, 0.0, ST,
+                                   C.byref(g)) == 0
+        return g
+    g = graph()
+    for seen, rc in ((dict(flags=1), INVALID), (dict(flags=2), INVALID), (dict(flags=4), INVALID),
+                     (dict(flags=8), INVALID), (dict(radial=1 << 31), -4), (dict(angular=1 << 31), -4)):
+        found(**seen)
+        assert L.gnep_rebuild_neighbors(m, C.byref(b), nl, ST) == rc, seen
+        assert L.gnep_graph_launch(g, ST) == 0, seen
+    found()
+    assert L.gnep_rebuild_neighbors(m, C.byref(b), nl, ST) == 0
+    assert L.gnep_graph_launch(g, ST) == INVALID
+    g = graph()
+    found(flags=8)  # positions that are not numbers after the drift
+    F = device([0.0] * 6, "f")
+    pos, vel, im = device([1.0] * 6, "d"), device([0.0] * 6, "d"), device([1.0, 1.0], "d")
+    assert L.gnep_md_verlet(m, nl, pos, vel, im, F, 1.0, None, ST) == INVALID
+    assert L.gnep_graph_launch(g, ST) == INVALID
+    """)
