@@ -39,6 +39,16 @@ bool gnep::is_device_ptr(const void* p) {
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+bool gnep::kernel_can_use(const void* p, size_t align, int device) {
+  cudaPointerAttributes a;
+  if (!p || reinterpret_cast<uintptr_t>(p) % align != 0) return false;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == device);
+}
+
 namespace {
 
 // Copy to a caller buffer (host or device); host destinations are complete on return.
@@ -460,9 +470,9 @@ int gnep_forward(gnep_model* m, const gnep_nlist* nl_, float* E_atom, double* E_
   gnep_nlist* nl = const_cast<gnep_nlist*>(nl_);
   cudaStream_t st = (cudaStream_t)stream;
   StepArgs A{m, nl, st};
-  // device buffers are written by the last kernel, host ones copied below
-  A.out = {is_device_ptr(E_atom) ? E_atom : nullptr, is_device_ptr(F) ? F : nullptr,
-           is_device_ptr(E_struct) ? E_struct : nullptr, is_device_ptr(W_struct) ? W_struct : nullptr};
+  // this GPU's buffers are written by the last kernel, others copied to below
+  auto direct = [&](auto* p) { return kernel_can_use(p, sizeof(*p), nl->device) ? p : nullptr; };
+  A.out = {direct(E_atom), direct(F), direct(E_struct), direct(W_struct)};
   if ((rc = run_descriptors(A, true))) return rc;
   if ((rc = run_forward(A))) return rc;
   const size_t N = nl->n_atoms, S = nl->n_struct;
@@ -484,7 +494,7 @@ int gnep_md_verlet(gnep_model* m, gnep_nlist* nl, double* pos, double* vel, cons
   if ((rc = md_kick_drift(nl, pos, vel, inv_mass, F, dt, st))) return rc;  // leaves the positions in the list too
   if ((rc = finish_build(m, nl, nullptr, st, false))) return rc;           // lists for the new positions
   StepArgs A{m, nl, st};
-  A.out.Es = is_device_ptr(E_struct) ? E_struct : nullptr;
+  A.out.Es = kernel_can_use(E_struct, 8, nl->device) ? E_struct : nullptr;
   if ((rc = run_descriptors(A, true))) return rc;
   if ((rc = run_forward(A))) return rc;
   if ((rc = md_kick(nl, vel, inv_mass, F, dt, st))) return rc;  // leaves the forces in F

@@ -199,6 +199,9 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
 // neighbors.cu
 int build_lists(gnep_model* m, gnep_nlist* nl, const gnep_batch* b, cudaStream_t st, bool* types_changed);
 bool is_device_ptr(const void* p);  // api.cu
+// Whether a kernel on `device` may read or write p itself: device memory of that GPU
+// or managed memory, aligned for its type.  Anything else takes a copy (api.cu).
+bool kernel_can_use(const void* p, size_t align, int device);
 
 // Shape-specialised step (sweeps.cu).
 struct StepArgs {

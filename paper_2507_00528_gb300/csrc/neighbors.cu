@@ -978,8 +978,9 @@ int build_lists(gnep_model* m, gnep_nlist* nl, const gnep_batch* b, cudaStream_t
   Slots sl;  // one pass into per-atom slots; atoms with more neighbours take the batch to a second, writing pass
   sl.cap = kSlots;
   // zeroed: result, bin counts and cursors; then the rest
-  const bool stage = b && !(is_device_ptr(b->struct_off) && is_device_ptr(b->type) && is_device_ptr(b->pos) &&
-                            is_device_ptr(b->cell));  // host arrays are copied over first
+  // host arrays, and what the kernels must not read in place, are copied over first
+  const bool stage = b && !(kernel_can_use(b->struct_off, 4, nl->device) && kernel_can_use(b->type, 4, nl->device) &&
+                            kernel_can_use(b->pos, 8, nl->device) && kernel_can_use(b->cell, 8, nl->device));
   struct Item { void** p; size_t bytes; };
   const Item items[] = {
       {(void**)&A.res, sizeof(BuildResult)}, {(void**)&A.bcount, 4 * n}, {(void**)&A.bcursor, 4 * n},

@@ -1,7 +1,7 @@
 """What a list and the graphs captured on it keep over rebuilds: a rebuild on a side
 stream into a batch with many more pairs (lists and workspace grow), evaluated at once
 on that stream, against a list built anew; and training graphs over rebuilds that are
-refused."""
+refused; and what an evaluation leaves in host and device outputs."""
 import numpy as np
 import pytest
 import torch
@@ -68,3 +68,22 @@ def test_training_graph_outlives_a_refused_rebuild(what):
     c.nl.rebuild(gnep.DeviceBatch.from_host(b))
     with pytest.raises(gnep._lib.GnepError, match="rebuilt or retuned"):
         g.launch()
+
+
+def test_outputs_to_host_and_device_agree():
+    b = small_cells_batch()
+    c = Case("nmax4_basis8_h30", b, labels=False)
+    dev = c.m.forward(c.nl)
+    host = [np.full(tuple(t.shape), -1.0, dtype=np.float32 if t.dtype == torch.float32 else np.float64) for t in dev]
+    st = torch.cuda.current_stream().cuda_stream
+    L = gnep._lib.load()
+    gnep.check(L.gnep_forward(c.m.h, c.nl.h, *(h.ctypes.data for h in host), st))
+    for d, h in zip(dev, host):
+        np.testing.assert_array_equal(d.cpu().numpy(), h)
+    # two outputs in host memory and two on the device, one of them off its alignment
+    raw = torch.zeros(4 * b.n_atoms * 3 + 8, dtype=torch.uint8, device="cuda")
+    Es, W = np.zeros(b.n_struct), torch.zeros(b.n_struct, 6, dtype=torch.float64, device="cuda")
+    gnep.check(L.gnep_forward(c.m.h, c.nl.h, None, Es.ctypes.data, raw.data_ptr() + 2, W.data_ptr(), st))
+    torch.cuda.synchronize()
+    F = raw[2:2 + 4 * b.n_atoms * 3].cpu().numpy().tobytes()
+    assert F == host[2].tobytes() and (Es == host[1]).all() and (W.cpu().numpy() == host[3]).all()

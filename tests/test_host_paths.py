@@ -185,3 +185,44 @@ def test_a_refused_batch_leaves_captured_graphs(run):
     assert L.gnep_md_verlet(m, nl, pos, vel, im, F, 1.0, None, ST) == INVALID
     assert L.gnep_graph_launch(g, ST) == INVALID
     """)
+
+
+def test_buffers_that_kernels_must_not_touch_are_copied(run):
+    """Batch arrays and outputs in this GPU's memory are used in place; in another GPU's,
+    or off their type's alignment, they are copied."""
+    run("""
+    m, b = model(), batch()
+    nl = built(m, b)
+    names = ("struct_off", "pos", "type", "cell")
+    assert [fake.fake_copies(getattr(b, f)) for f in names] == [0] * 4
+    for f in names:
+        other = batch()
+        fake.fake_foreign(getattr(other, f))
+        found()
+        assert L.gnep_rebuild_neighbors(m, C.byref(other), nl, ST) == 0
+        assert fake.fake_copies(getattr(other, f)) == 1, f
+    for f, values, fmt in (("pos", [1.0] * 6, "d"), ("cell", [9.0] * 9, "d"), ("type", [0, 1], "i")):
+        other, room = batch(), device([0] * 100, "b")
+        at = room + (4 if fmt == "d" else 2)
+        C.memmove(at, struct.pack("%d%s" % (len(values), fmt), *values), 4 * len(values))
+        setattr(other, f, at)
+        found()
+        assert L.gnep_rebuild_neighbors(m, C.byref(other), nl, ST) == 0
+        assert fake.fake_copies(at) == 1, f
+    sizes = (("f", 2), ("d", 1), ("f", 6), ("d", 6))
+    for k in range(4):
+        for foreign, shift in ((False, 0), (True, 0), (False, 2)):
+            out = [device([0.0] * (n + 1), t) for t, n in sizes]
+            out[k] += shift
+            if foreign:
+                fake.fake_foreign(out[k])
+            assert L.gnep_forward(m, nl, *out, ST) == 0
+            assert [fake.fake_copies(p) for p in out] == [int(q == k and (foreign or shift > 0)) for q in range(4)]
+    F = device([0.0] * 6, "f")
+    pos, vel, im, E = device([1.0] * 6, "d"), device([0.0] * 6, "d"), device([1.0, 1.0], "d"), device([0.0], "d")
+    for copies in (0, 1):
+        found()
+        assert L.gnep_md_verlet(m, nl, pos, vel, im, F, 1.0, E, ST) == 0
+        assert fake.fake_copies(E) == copies
+        fake.fake_foreign(E)
+    """)
