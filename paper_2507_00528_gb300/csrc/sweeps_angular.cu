@@ -89,11 +89,11 @@ __device__ __forceinline__ void write_pair_row(float* row, const float* cIJ, flo
       constexpr int l = decltype(lc)::value, q0 = l * l - 1;
 #pragma unroll
       for (int k = 0; k <= 2 * l; ++k) B[q0 + k] = solid_comp(R, k);
-      if constexpr (TAN) {
+      if constexpr (TAN) {  // grad B . w = grad R . (w - (u . w) u) / r
         float d[2 * l + 1];
-        solid_dir<l>(L, w.x, w.y, w.z, d);
+        solid_dir<l>(L, (w.x - ru * ux) * ri, (w.y - ru * uy) * ri, (w.z - ru * uz) * ri, d);
 #pragma unroll
-        for (int k = 0; k <= 2 * l; ++k) D[q0 + k] = fmaf(-(float)l * ru, B[q0 + k], d[k]) * ri;
+        for (int k = 0; k <= 2 * l; ++k) D[q0 + k] = d[k];
       }
       flush(std::integral_constant<int, q0>{}, std::integral_constant<int, q0 + 2 * l + 1>{});
     });
@@ -648,11 +648,10 @@ __global__ void __launch_bounds__(32 * kAngW, C::LMAX > 4 ? 3 : 4)
           solid_levels<C::LMAX>(ux, uy, uz, [&](auto lc, const auto& Rl, const auto& Ll) {
             constexpr int l = decltype(lc)::value;
             float d[2 * l + 1];
-            solid_dir<l>(Ll, w.x, w.y, w.z, d);
+            solid_dir<l>(Ll, (w.x - ru * ux) * ri, (w.y - ru * uy) * ri, (w.z - ru * uz) * ri, d);
 #pragma unroll
             for (int k = 0; k <= 2 * l; ++k) {
-              const float bq = solid_comp(Rl, k);
-              const float2 b2 = dup2(bq), d2 = dup2(fmaf(-(float)l * ru, bq, d[k]) * ri);
+              const float2 b2 = dup2(solid_comp(Rl, k)), d2 = dup2(d[k]);
               float s[R::HW];
               load_row4<R::HW / 4>(hr + (l * l - 1 + k - NLM) * R::HW, s);
 #pragma unroll
