@@ -712,11 +712,10 @@ bool radial_beside(const gnep_nlist* nl) {
 
 // Persistent blocks of the c-gradient sweep: enough warps for every atom group
 // up to the default (or tuned) count, at most kCgBlocksMax (the size of the
-// partial buffer).  The default is what an SM holds: four blocks, three at
-// l_max > 4.
+// partial buffer).  The default is what the SMs hold.
 int cgrad_blocks(const gnep_nlist* nl) {
   const int per = ang_block_atoms(nl->shape), need = (nl->n_atoms + per - 1) / per;
-  int cap = nl->tune.cg_blocks > 0 ? nl->tune.cg_blocks : (nl->shape.lmax > 4 ? 3 : 4) * sm_count();
+  int cap = nl->tune.cg_blocks > 0 ? nl->tune.cg_blocks : ang_cgrad_per_sm(nl->shape.lmax) * sm_count();
   if (cap > kCgBlocksMax) cap = kCgBlocksMax;
   return need < cap ? (need > 0 ? need : 1) : cap;
 }

@@ -263,6 +263,7 @@ __global__ void __launch_bounds__(32 * kAngW, TAN ? (C::LMAX > 4 || C::NQA < 9 ?
       });
     }
     if constexpr (C::FB) {
+      static_assert(A::QG >= TN, "a lane per row of the tile");
       float y2[5], v;
       spread_moments<C>(y, lane, qg, y2);
       if constexpr (TAN) {
@@ -370,7 +371,7 @@ __global__ void __launch_bounds__(32 * kAngW)
         float e[C::LMAX + 1];
 #pragma unroll
         for (int l = lb; l <= ang_deg(base + NQL - 1); ++l) e[l] = 2.f * ep[C::vang(n, l)];
-float g4[5], e4 = 0.f;
+        float g4[5], e4 = 0.f;
         if constexpr (C::FB && base == 0) {
           q4_grad(&x[3], g4);
           e4 = ep[C::v4b(n)];
@@ -499,7 +500,7 @@ struct CgradRow {
 };
 
 template <class C>
-__global__ void __launch_bounds__(32 * kAngW, C::LMAX > 4 ? 3 : 4)
+__global__ void __launch_bounds__(32 * kAngW, ang_cgrad_per_sm(C::LMAX))
     k_ang_cgrad(int N, DevModel dm, const int* __restrict__ type, const int* __restrict__ off,
                 const float4* __restrict__ rij, const float4* __restrict__ wij, const float* __restrict__ S,
                 const float* __restrict__ Sd, const float* __restrict__ Gb, const float* __restrict__ Ep,
@@ -736,7 +737,7 @@ int resident(K kern, size_t smem, int& cap) {
 // Resident blocks per kernel (the same value on every model creation).
 template <class C>
 struct Caps {
-  inline static int desc = 0, tangent = 0, force = 0, cgrad = 0;
+  inline static int desc = 0, tangent = 0, force = 0;
 };
 
 template <class C>
@@ -756,7 +757,8 @@ int ang_setup() {
   if (int rc = resident(k_ang_desc<C, false>, DescRow<C, false>::smem, Caps<C>::desc)) return rc;
   if (int rc = resident(k_ang_desc<C, true>, DescRow<C, true>::smem, Caps<C>::tangent)) return rc;
   if (int rc = resident(k_ang_force<C>, ForceRow<C>::smem, Caps<C>::force)) return rc;
-  return resident(k_ang_cgrad<C>, CgradRow<C>::smem, Caps<C>::cgrad);
+  int cgrad = 0;  // its grid is cgrad_blocks
+  return resident(k_ang_cgrad<C>, CgradRow<C>::smem, cgrad);
 }
 
 template <class C>

@@ -10,6 +10,8 @@ namespace gnep {
 
 // Atoms of one block of the angular sweeps (four warps, a group of atoms each).
 int ang_block_atoms(const Shape& s);
+// Blocks of the c-gradient sweep per SM: what its registers are bounded for, and its grid.
+constexpr int ang_cgrad_per_sm(int lmax) { return lmax > 4 ? 3 : 4; }
 
 template <class C>
 int ang_setup();

@@ -46,10 +46,9 @@ struct LossArgs {
 // coef[0..3] = {L, L_e, L_f, L_v}; coef[4] = cf, coef[5] = ce, coef[6] = cv with
 //   a_i = cf (F_i - F_i^tar),  e_s = ce (E_s/N_s - E_s^tar)/N_s,
 //   B_s = cv (W_s/N_s - V_s^tar)/N_s  (off-diagonals halved).
-// l2p: the parts of sum theta^2, one per structure (NULL: summed here).
+// l2p: the parts of sum theta^2, one per structure (NULL without the L2 term).
 __device__ void loss_final_block(const LossArgs& a, int nred, const double* __restrict__ red,
-                                 const double* __restrict__ l2p, const float* __restrict__ params,
-                                 double* __restrict__ coef, int* __restrict__ err) {
+                                 const double* __restrict__ l2p, double* __restrict__ coef, int* __restrict__ err) {
   __shared__ double sh[32 * 4];
   __shared__ double tot[4], root[3], chain[3];
   double v[4] = {0.0, 0.0, 0.0, 0.0};
@@ -59,8 +58,6 @@ __device__ void loss_final_block(const LossArgs& a, int nred, const double* __re
     v[2] += red[3 * b + 2];
     if (l2p) v[3] += l2p[b];
   }
-  if (a.l2 != 0.0 && !l2p)
-    for (int64_t q = threadIdx.x; q < a.n_params; q += blockDim.x) v[3] += (double)params[q] * params[q];
   const double r = block_sums<4>(v, sh);
   if (threadIdx.x < 4) {
     const double L = r * (threadIdx.x == 0 ? a.inv_S : threadIdx.x == 1 ? a.inv_3N : threadIdx.x == 2 ? a.inv_6S : 1.0);
@@ -91,13 +88,6 @@ __device__ void loss_final_block(const LossArgs& a, int nred, const double* __re
   coef[5] = 2.0 * a.le * ke * a.inv_S;   // Eq. 14
   coef[6] = 2.0 * a.lv * kv * a.inv_6S;  // Eq. 16
   if (!isfinite(L)) atomicOr(err, kErrNonFinite);
-}
-
-__global__ void __launch_bounds__(256) k_loss_final(LossArgs a, int nred, const double* __restrict__ red,
-                                                    const float* __restrict__ params, double* __restrict__ coef,
-                                                    int* __restrict__ err) {
-  GNEP_PDL_START();
-  loss_final_block(a, nred, red, nullptr, params, coef, err);
 }
 
 // Per structure s (one block of 128 threads): the sums E_s and W_s (Eqs. 1, 4)
@@ -204,7 +194,7 @@ __global__ void __launch_bounds__(128) k_struct_loss(const int* __restrict__ sof
   __syncthreads();
   if (!last) return;
   __threadfence();
-  loss_final_block(la, (int)gridDim.x, red, la.l2 != 0.0 ? l2p : nullptr, params, coef, err);
+  loss_final_block(la, (int)gridDim.x, red, la.l2 != 0.0 ? l2p : nullptr, coef, err);
   if (threadIdx.x == 0 && gridDim.x > 1) *done = 0;
 }
 
@@ -499,19 +489,16 @@ int run_loss_impl(const gnep_model* m, gnep_nlist* nl, const double* le, const f
   LossArgs a;
   a.N = N; a.S = S; a.le = y->lambda_e; a.lf = y->lambda_f; a.lv = y->lambda_v; a.l2 = y->lambda_l2;
   a.form = y->loss_form; a.n_params = m->n_params;
-  a.inv_S = S > 0 ? 1.0 / S : 0.0;
-  a.inv_3N = N > 0 ? 1.0 / (3.0 * N) : 0.0;
-  a.inv_6S = S > 0 ? 1.0 / (6.0 * S) : 0.0;
+  a.inv_S = 1.0 / S;  // a batch holds a structure, and a structure an atom
+  a.inv_3N = 1.0 / (3.0 * N);
+  a.inv_6S = 1.0 / (6.0 * S);
   a.inv_np = 1.0 / (double)m->n_params;
-  if (S > 0) {  // per-structure residuals; the last block forms the loss terms
-    (void)launch_pdl(k_struct_loss, S, 128, 0, st, nl->struct_off, w.Eatom, w.Wat, w.F, le, lf, lv, w.Es, w.Ws, w.red,
-                                     w.red + 3 * (size_t)S, w.red + 10 * (size_t)S, a, m->params, w.coef, m->err, m->err + 2, w.a, w.es,
-                                     w.Bs);
-  } else {
-    (void)launch_pdl(k_loss_final, 1, 256, 0, st, a, 0, w.red, m->params, w.coef, m->err);
-  }
+  // per-structure residuals; the last block forms the loss terms
+  (void)launch_pdl(k_struct_loss, S, 128, 0, st, nl->struct_off, w.Eatom, w.Wat, w.F, le, lf, lv, w.Es, w.Ws, w.red,
+                   w.red + 3 * (size_t)S, w.red + 10 * (size_t)S, a, m->params, w.coef, m->err, m->err + 2, w.a, w.es,
+                   w.Bs);
   stage("struct_loss");
-  if (N + S > 0 && (S == 0 || a.form == GNEP_LOSS_RMSE)) {  // the loss kernel wrote them in the MSE form
+  if (a.form == GNEP_LOSS_RMSE) {  // the loss kernel wrote them in the MSE form
     (void)launch_pdl(k_residuals, blocks_for(N + S, 256), 256, 0, st, N, S, w.F, lf, w.red + 3 * (size_t)S, w.coef, w.a, w.es,
                                                          w.Bs);
     stage("residuals");
