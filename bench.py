@@ -4,10 +4,10 @@
 One step = the whole hot path over one batch: descriptors, network, energies,
 forces, virials, loss, the exact gradient w.r.t. every parameter, and an Adam
 update with the Eq. 17 learning rate, captured once as a CUDA graph and
-replayed.  The headline runs the FP32 form (FP32 network; the sweep
-contractions as split-TF32 tensor-core products with FP32-level error, held
-to the FP32 tolerances against the FP64 oracle); the BF16 and TF32 network
-modes are timed beside it with their force difference from it.  The workload
+replayed.  The headline runs the FP32 form (sweeps as FP32 multiply-adds; the
+network as split-TF32 tensor-core products added in FP32, with FP32-level
+error; all held to the FP32 tolerances against the FP64 oracle); the BF16 and
+TF32 network modes are timed beside it with their force difference from it.  The workload
 is 256 synthetic Sb/Te structures of 32-400 atoms (perturbed rocksalt,
 liquid-like and strained cells in equal thirds), n_max 8/8, basis 12/12,
 l_max 4 with the 4-body term, 50 hidden neurons, labels from a random teacher
@@ -87,7 +87,7 @@ def work_model_flops(nqr=9, kr=13, nqa=9, ka=13, ns=2, H=50, fb=True, N=1, PR=1,
     return f
 
 
-def algo_bytes(nqr=9, kr=13, nqa=9, ka=13, ns=2, H=50, fb=True, N=1, PR=1, PA=1, HP=64):
+def algo_bytes(nqr=9, kr=13, nqa=9, ka=13, ns=2, H=50, fb=True, N=1, PR=1, PA=1):
     """Compulsory DRAM bytes per launch of each kernel: every input the
     kernel needs read once and every output written once (FP32 arrays, int32
     indices, float4 pair vectors), nothing re-read."""
@@ -98,12 +98,12 @@ def algo_bytes(nqr=9, kr=13, nqa=9, ka=13, ns=2, H=50, fb=True, N=1, PR=1, PA=1,
     b = {}
     b["desc_radial"] = 4 * (PR * 4 + 2 * N + N * FRn + N * nqr)
     b["desc_angular"] = 4 * (PA * 4 + 2 * N + N * A + N * ang_cols)
-    b["mlp_fwd"] = 4 * N * (D + D + 1 + HP + FRn)
-    b["force_angular"] = 4 * (PA * 5 + N * A + N * D + PA * 4)
+    b["mlp_fwd"] = 4 * N * (D + D + 1 + FRn)
+    b["force_angular"] = 4 * (PA * 4 + N * A + N * D + PA * 4)
     b["force_atoms"] = 4 * (PR * 5 + N * FRn + N + PA * 9 + 9 * N)
     b["tangent_radial"] = 4 * (PR * 5 + 4 * N + N * FRn + N * nqr)
     b["tangent_angular"] = 4 * (PA * 6 + 4 * N + N * A + N * A + N * ang_cols + PA * 4)
-    b["mlp_bwd"] = 4 * N * (2 * D + HP + D + 2)
+    b["mlp_bwd"] = 4 * N * (2 * D + D + 2)
     b["cgrad"] = 4 * (N * (2 * A + 2 * (ang_cols + nqr)) + PA * 8 + N)
     b["cgrad_radial"] = 4 * N * (2 * nqr + 2 * FRn + 1)
     return b
@@ -461,7 +461,7 @@ def run_gnep(args):
 
 
 DTYPES = {
-    "fp32": "f32 (FP32 geometry and network; descriptor, force, tangent and c-gradient contractions as "
+    "fp32": "f32 (FP32 geometry and descriptor, force, tangent and c-gradient contractions; network as "
             "split-TF32 tensor-core products with FP32-level error; FP64 cross-atom sums)",
     "tf32": "tf32 network (tcgen05, FP32 accumulation); otherwise as the f32 form",
     "bf16": "bf16 network (tcgen05, FP32 accumulation); otherwise as the f32 form",

@@ -3,7 +3,7 @@
  *
  * The library evaluates, for a packed batch of periodic structures, the NEP
  * descriptor (radial Chebyshev terms, Eqs. 5-6 with App. A; angular terms from
- * real solid harmonics with l <= 4, Eqs. 7-8 with App. B; an optional 4-body
+ * real solid harmonics with l <= 8, Eqs. 7-8 with App. B; an optional 4-body
  * term), a one-hidden-layer tanh network per element (D1.1), energies, forces
  * and virials (Eqs. 1, 3, 4), the weighted energy/force/virial loss (Eqs. 9-12)
  * and its exact gradient with respect to every network weight and descriptor
@@ -54,12 +54,15 @@ typedef enum {
   GNEP_ERR_UNSUPPORTED = -8        /* hyper-parameters without a compiled kernel */
 } gnep_status;
 
-/* Arithmetic of the network contractions (D1.1-D1.10) only.  FP32: CUDA-core
- * FP32.  TF32 / BF16: tcgen05 tensor-core products with TF32 / BF16 operands
- * and FP32 accumulation.  In every mode the per-pair geometry is FP32, the
- * descriptor, force, tangent and coefficient-gradient contractions are
- * FP32-accurate (split-TF32 tensor-core products), and the cross-atom sums of
- * energies, virials, loss and gradient are FP64 above FP32 leaves. */
+/* Arithmetic of the network contractions (D1.1-D1.10) only.  FP32: products of
+ * operands split into two TF32 parts (hi hi + hi lo + lo hi, about 22 bits) on
+ * warp-level tensor cores, added in FP32; against FP64 they err about as much as
+ * chains of FP32 multiply-adds (gradients of small batches 1.3e-7 against
+ * 1.4e-7).  TF32 / BF16: tcgen05 tensor-core products with TF32 / BF16 operands
+ * and FP32 accumulation.  In every mode the per-pair geometry and the
+ * descriptor, force, tangent and coefficient-gradient contractions are FP32
+ * multiply-adds, and the cross-atom sums of energies, virials, loss and gradient
+ * are FP64 above FP32 leaves. */
 enum { GNEP_PREC_FP32 = 0, GNEP_PREC_TF32 = 1, GNEP_PREC_BF16 = 2 };
 /* GNEP_LOSS_MSE: Eq. 9 with Eqs. 10-12.  GNEP_LOSS_RMSE: the same weighted sum
  * of the square roots of Eqs. 10-12. */
@@ -185,7 +188,7 @@ int gnep_descriptors(gnep_model *m, const gnep_nlist *nl, float *G, void *stream
  * the library holds it until the process exits) instead of the nlist's
  * workspace.  A batch fits when
  *   roundup64(n_atoms * n_species * (basis_radial + 1))
- *     + n_atoms * 24 * (n_max_angular + 1)  <=  2^21 floats
+ *     + n_atoms * ((l_max + 1)^2 - 1) * (n_max_angular + 1)  <=  2^21 floats
  * (roundup64: the next multiple of 64); larger batches return INVALID_ARG.
  * G [n_atoms][N_des] must be device memory; it is written asynchronously on
  * `stream` after the nlist's last build.  The first call on each device looks

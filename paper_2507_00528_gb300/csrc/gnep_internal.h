@@ -85,15 +85,16 @@ struct gnep_nlist {
   int* perm = nullptr;         // device [N] atoms grouped by species
   int species_off[9] = {0};    // host [ns+1]
   gnep::PairList L[2];         // radial, angular
-  // Launch shapes chosen by gnep_autotune (0 = built-in default): atoms and
-  // pairs per tile of each tile set, persistent blocks of the c-gradient sweep
-  // and of the network kernels, lanes per atom of the radial sweeps (4, 8, 16),
-  // atoms per FP32 network tile (32, 128) and where the radial sweeps run
+  // Launch shapes chosen by gnep_autotune (0 = built-in default): na and ch, the
+  // tile limits of earlier angular sweeps (kept for gnep_tuning_get, no kernel
+  // reads them), persistent blocks of the c-gradient sweep and of the network
+  // kernels, lanes per atom of the radial sweeps (4, 8, 16), atoms per FP32
+  // network tile (32; 128 for two tiles of 64) and where the radial sweeps run
   // (1: in turn with the angular ones, 2: beside them on the second stream).
   struct Tuning {
     int na[2] = {0, 0}, ch[2] = {0, 0}, cg_blocks = 0, net_blocks = 0, radial_lanes = 0, net_tile = 0, beside = 0;
   } tune;
-  uint64_t gen = 0;  // bumped whenever lists or tiles change (captured graphs check it)
+  uint64_t gen = 0;  // bumped whenever lists or launch shapes change (captured graphs check it)
   bool built = false;        // lists, species grouping and workspace belong to one batch (false after a failed build)
   int last_err = 0;          // the model's error flag as the last build's search saw it
   void* host_res = nullptr;  // pinned: what a build's search reports to the host
@@ -165,7 +166,7 @@ int cuda_error(cudaError_t e, const char* what);
     if (cond) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");        \
   } while (0)
 #define GNEP_PDL_START() GNEP_PDL_START_IF(gridDim.x * blockDim.x <= gnep::kPdlThreads)
-constexpr unsigned kPdlThreads = 768 * 152;
+constexpr unsigned kPdlThreads = 768 * 152;  // GB300 has 152 SMs; a constant, since kernels read it
 
 // launch_on launches as a dependent of the stream's previous kernel when `pdl`
 // is set, else as an ordinary launch.

@@ -584,7 +584,7 @@ __device__ __forceinline__ void pairs_flat(const BuildArgs& A, const ListParams&
 
 // Binned search, one warp per central atom i (the slot pass) of the
 // structures above kCellMinAtoms atoms; the smaller ones take the all-pairs
-// search (k_pairs_flat), which is as fast there: at cell widths below 3 r_c the
+// search (pairs_flat), which is as fast there: at cell widths below 3 r_c the
 // visited bins cover about the whole cell.  The bins of structure s split its
 // cell into nbin[s] parts along each cell direction; every (j, n) within r_c of
 // i has f_j + n inside (f_i - t, f_i + t) along each direction (t = r_c / w_x,
@@ -676,9 +676,9 @@ __device__ __forceinline__ void pairs_cell(const BuildArgs& A, const ListParams&
 // a neighbour has one image that can be within r_c, n = -round(f_j - f_i), so each
 // lane tests its j there, two j per lane and round, with the decision of the other
 // searches.  Most structures of training batches are such cells; laying their
-// (j, image) candidates out as below took half as long again (256 structures of
-// 32-400 atoms: k_pairs_slots 122 us, now 80; instruction issue bounds it, 72 % of
-// the issue slots).
+// (j, image) candidates out as for narrower cells took half as long again (256
+// structures of 32-400 atoms: k_pairs_slots 130 us, now 93; 57 % of the issue slots,
+// the rest waits on the loads of phi and frac).
 __device__ __forceinline__ void pairs_min(const BuildArgs& A, const ListParams& lp, const Slots& sl, int i, int s,
                                           int lane) {
   const int a0 = A.off[s], a1 = A.off[s + 1];
@@ -964,8 +964,8 @@ __global__ void k_reverse(int64_t P, const int* __restrict__ off, const int* __r
 // k_offsets, the wait, k_compact, k_reverse.  What bounds a small build is this
 // chain and the wait, not work: with a launch per check, scan level, conversion
 // and copy, 14 allocations, and tiles cut on the host, rebuilding and evaluating
-// one structure of 139 atoms took 310 us, now 143; 256 structures 757, now 365; a
-// molecular dynamics step of 4,096 atoms 316, now 152.
+// one structure of 139 atoms took 310 us, now 137; 256 structures 757, now 364; a
+// molecular dynamics step of 4,096 atoms 316, now 146.
 int build_lists(gnep_model* m, gnep_nlist* nl, const gnep_batch* b, cudaStream_t st, bool* types_changed) {
   const int N = nl->n_atoms, S = nl->n_struct;
   BuildArgs A;

@@ -727,8 +727,9 @@ int cgrad_radial_blocks(const gnep_nlist* nl) {
   return nb < fit ? nb : fit;
 }
 
-// Default tile limits of the tuning interface: [0] 32 atoms and 256 pairs, [1] 128
-// / channels and 128 pairs.  The angular sweeps cut no tiles any more.
+// What gnep_tuning_get reports for the values 0 to 3 by default: the tile limits of
+// earlier angular sweeps ([0] 32 atoms and 256 pairs, [1] 128 / channels and 128
+// pairs).  The present ones cut no tiles.
 void angular_tile_limits(const Shape& s, int which, int* na, int* ch) {
   const int nq = s.nqr > s.nqa ? s.nqr : s.nqa;
   if (which == 0) {

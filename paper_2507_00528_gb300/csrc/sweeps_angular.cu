@@ -129,7 +129,7 @@ __device__ __forceinline__ void degree_sums(const float (&t)[8], int qg, F&& emi
 // (stored for sweep 4) Sdot_nq = sum_j [g_n' (u . w) B_q + g_n D_q],
 // qdot_nl = 2 sum_m C S Sdot and the 4-body tangent.
 // Bound by shared-memory bandwidth and the latency of a warp's alternating
-// phases (ncu: 65% of the wavefront slots, issue slots 45% used).  Three atoms a
+// phases (ncu: 64 to 68% of the wavefront slots, a third of the issue slots used).  Three atoms a
 // warp, because their 25 pairs and 27 summing lanes fill both mappings; a summing
 // lane's 3 x 8 tile reads 11 values for 24 products (one channel of all 24
 // components: 25 for 24).  On the 256-structure batch (55,200 atoms, 460,534
@@ -137,6 +137,9 @@ __device__ __forceinline__ void degree_sums(const float (&t)[8], int qg, F&& emi
 // us (one channel per lane: 40 and 65; per-atom split-TF32 tensor-core tiles: 68
 // and 106); at l_max 8 43 and 102 us (61 and 121; lanes summing one (n,
 // component) each over the pairs: 464 and 711).
+// Blocks per SM: the register bound at which a thread spills at most 104 bytes; one
+// block more spills 108 to 288 bytes in the tangent, and 20 to 60 in the descriptors
+// (but for l_max 6), where now at most 4 do.
 template <class C, bool TAN>
 __global__ void __launch_bounds__(32 * kAngW, TAN ? (C::LMAX > 4 || C::NQA < 9 ? 3 : 4) : (C::LMAX > 4 ? 4 : 5))
     k_ang_desc(int N, DevModel dm, const int* __restrict__ type, const int* __restrict__ atom_struct,
@@ -328,7 +331,7 @@ __device__ __forceinline__ void load_row4(const float* p, float (&x)[4 * N4]) {
 //   ghat_q = sum_n g_n Shat_nq,  ghat'_q = sum_n g_n' Shat_nq,
 //   Shat_nq = dE_i/dS_nq = 2 C_q E'_{n l} S_nq (+ E'_4b,n dq4/dS_n2m).
 // Channel lanes form Shat in shared memory, pair lanes contract it.  Bound by
-// shared-memory bandwidth (216 row values and 144 coefficients per pair at
+// shared-memory bandwidth (216 row values and 120 coefficients per pair at
 // n_max 8).  256 structures: 42 us at n_max 8, l_max 4, against 48 us with block
 // tiles and the gradient of every component projected; 73 us at l_max 8 against
 // 480 us with three lanes per pair running the recurrence in dual numbers.
@@ -481,9 +484,9 @@ __global__ void __launch_bounds__(32 * kAngW)
 // registers over all of a warp's groups; the block folds its warps in order and
 // writes cpart[block][c^A] once.  Bound by shared-memory bandwidth (each pair
 // lane reads its atom's 432 row values, 27 output lanes 12 values per pair).
-// 256 structures: 94 us at n_max 8, l_max 4, against 125 us as split-TF32
-// tensor-core products in block tiles; 178 us at n_max 4, l_max 8, against 770
-// us with a pair per lane and scalar row loads.
+// 256 structures: 91 us at n_max 8, l_max 4 (71% of the wavefront slots), against
+// 125 us as split-TF32 tensor-core products in block tiles; 143 us at n_max 4,
+// l_max 8, against 770 us with a pair per lane and scalar row loads.
 template <class C>
 struct CgradRow {
   using A = Ang<C>;

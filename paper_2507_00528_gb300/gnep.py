@@ -133,7 +133,7 @@ class NeighborList:
                    "net_blocks", "radial_lanes", "net_tile_atoms", "radial_beside")
 
     def autotune(self, y: "Labels", reps: int = 3, stream=None) -> dict:
-        """Pick the fastest launch shapes of the angular sweeps for this batch
+        """Pick the fastest launch shapes of the sweeps and the network for this batch
         (times loss + gradient; invalidates graphs captured on this list)."""
         yc = y.c()
         check(_lib.load().gnep_autotune(self.model.h, self.h, C.byref(yc), reps, _stream(stream)))
@@ -145,7 +145,7 @@ class NeighborList:
         return dict(zip(self.TUNING_KEYS, v.tolist()))
 
     def set_tuning(self, values: dict | None = None, stream=None):
-        """Set launch shapes (missing or 0 = built-in default) and rebuild the tiles."""
+        """Set launch shapes (missing or 0 = built-in default); graphs captured on the list end."""
         values = values or {}
         v = np.array([int(values.get(k, 0)) for k in self.TUNING_KEYS], dtype=np.int32)
         check(_lib.load().gnep_tuning_set(self.model.h, self.h, v.ctypes.data, _stream(stream)))
